@@ -294,40 +294,6 @@ egm_status choose_band(const Plan &pl, const egm_params &prm, bool csr, int sms,
     return EGM_OK;
 }
 
-size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
-
-// Banded-form scratch: query permutation and buckets; with float pairs
-// (`packed`) also the sorted query records, the packed operand rows and
-// their norms (padded for the aligned 16-byte bulk copies that read past a
-// pair's last row).
-// Without float pairs the operand buffers keep one tile of rows, which the
-// band kernel's (unused) tensor maps cover.
-struct BandLayout {
-    size_t qperm, descA, descB, qbkt, qsrt, qscale, rnorm, fcand, fmask, qrank, qhist, part, part_n, arrived, total;
-    int64_t items;
-    BandLayout(int64_t nq, int64_t nr, int npairs, bool packed) {
-        const size_t rb = (size_t)band_row_bytes();
-        const int64_t ta = packed ? nq : band_tile_queries(), tb = packed ? nr : band_tile_queries();
-        qperm = 0;
-        descA = qperm + align256(sizeof(uint32_t) * (size_t)std::max<int64_t>(nq, 1));
-        descB = descA + align256(rb * (size_t)std::max<int64_t>(ta, 1));
-        qbkt = descB + align256(rb * (size_t)std::max<int64_t>(tb, 1));
-        qsrt = qbkt + align256(sizeof(uint16_t) * (size_t)std::max<int64_t>(nq, 1));
-        qscale = qsrt + align256(sizeof(QueryRec) * (size_t)std::max<int64_t>(packed ? nq : 1, 1));
-        rnorm = qscale + align256(sizeof(float) * (size_t)std::max<int64_t>(packed ? nq : 1, 1));
-        // 64 rows of padding: bulk copies of a 32-row box may run past the last row
-        fcand = rnorm + align256(sizeof(float4) * (size_t)((packed ? nr : 0) + 64));
-        fmask = fcand + align256(2 * sizeof(uint4) * (size_t)(packed ? nq : 0));
-        qrank = fmask + align256(sizeof(uint32_t) * (size_t)(packed ? nq : 0));
-        qhist = qrank + align256(sizeof(uint32_t) * (size_t)std::max<int64_t>(nq, 1));
-        items = std::min<int64_t>(kMaxSplit * (nq / band_tile_queries() + npairs), kSplitItems);
-        part = qhist + align256(sizeof(uint32_t) * (size_t)kQBuckets * kQPlacePairs);
-        part_n = part + align256(sizeof(ulonglong2) * (size_t)(items * band_tile_queries()));
-        arrived = part_n + align256(sizeof(uint32_t) * (size_t)(items * band_tile_queries()));
-        total = arrived + align256(sizeof(uint32_t) * (size_t)items);
-    }
-};
-
 cudaError_t reserve(Scratch &c_, int64_t nq, int64_t nr, int64_t ntab, int npairs, bool band, bool packed) {
     Scratch *c = &c_;
     cudaError_t e;

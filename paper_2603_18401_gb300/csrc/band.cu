@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(kQPlaceThreads) query_place_kernel(const __gri
 }
 
 // ------------------------------------------------------------ packing
-constexpr int kRowB = 256;  // packed operand row: 128 BF16 or 256 E4M3 values
+constexpr int kRowB = kBandRowBytes;  // packed operand row: 128 BF16 or 256 E4M3 values
 constexpr int kBinRowB = 32;  // binary row (256 bits), kept as it is
 
 // Float rows only (u8 and binary rows go to the band kernel as they are).
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(256) pack_kernel(Launch L) {
 }
 
 // ------------------------------------------------------------ band kernel
-constexpr int kTM = 128;                 // queries per tile (MMA M, TMEM lanes)
+constexpr int kTM = kBandTile;           // queries per tile (MMA M, TMEM lanes)
 constexpr int kBoxR = 32;                // reference rows per TMA box (N per box)
 constexpr int kBandThreads = kTM + 32;   // four epilogue warps and the control warp
 // Tile shapes (chosen per call regime by the tuner): CB boxes per MMA chunk

@@ -20,6 +20,7 @@
 #include <stdint.h>
 
 #include "../../include/egm.h"
+#include "band_layout.h"
 
 namespace egm {
 
@@ -141,6 +142,7 @@ struct __align__(16) QueryRec {
     int32_t pair;       // pair of this query
     uint32_t pad[2];
 };
+static_assert(sizeof(QueryRec) == kQueryRecBytes, "the banded scratch holds query records");
 
 // Queries per tile of the prefix sum of the candidate counts.
 constexpr int kCountTile = 4096;
@@ -186,7 +188,8 @@ struct Launch {
     uint32_t *qperm;              // sorted query slot -> pair-local query index
     uint16_t *qbkt;               // per query: its bucket of the angle order (written by the prep kernel)
     uint32_t *qhist;              // calls of up to kQPlacePairs pairs: queries in each bucket of each pair
-                                  //   (cleared by the geometry kernel, counted by the prep kernel)
+                                  //   (cleared by the geometry kernel while the previous call's last
+                                  //   kernel may still run, counted by the prep kernel)
     uint32_t *qrank;              //   and each query's rank in its bucket
     uint8_t *descA, *descB;       // float pairs: 256-byte operand rows of the sorted queries / references
     QueryRec *qsrt;               // float pairs: query records in sorted order, pad = (query index, norm
@@ -362,13 +365,7 @@ __device__ __forceinline__ bool exact_member(double a, double b, double c, doubl
 
 // Bucket of a query in the angle order of the banded form: the top bits of
 // its quantised line angle; lines without an FP32 view, or whose windows are
-// whole levels, after every angle.
-constexpr int kQSortBits = 11;
-constexpr int kQBuckets = (1 << kQSortBits) + 2;
-constexpr int kMaxSplit = 8;      // most items per tile of the banded form
-constexpr int64_t kSplitItems = 4096;  // most items of a call with split tiles
-constexpr int kQPlacePairs = 16;  // calls of up to so many pairs place the queries with several blocks a pair
-
+// whole levels, after every angle (kQBuckets in all, band_layout.h).
 __device__ __forceinline__ uint32_t query_bucket(const PairGeom &G, const QueryRec &r) {
     if (r.flags & EGM_FLAG_DEGENERATE_LINE) return 1u << kQSortBits;
     if ((r.flags & kQExactOnly) || (G.mode == kModeParallel && !(r.aux0 >= 0.5f))) return (1u << kQSortBits) + 1;

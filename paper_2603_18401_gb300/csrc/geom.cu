@@ -70,8 +70,9 @@ __global__ void __launch_bounds__(32) geometry_kernel(Launch L) {
         G.qkabs = 0u;
     }
 
-    // the counts of the queries' angle order (the previous call's are read
-    // before its band kernel starts)
+    // the counts of the queries' angle order: bytes that no call uses for
+    // anything else (band_layout.h), and the previous call's counts are read
+    // before its band kernel starts
     if (L.qhist)
         for (int b = lane; b < kQBuckets; b += 32) L.qhist[(int64_t)p * kQBuckets + b] = 0u;
 

@@ -218,8 +218,6 @@ __global__ void __launch_bounds__(128) gms_flag_kernel(const __grid_constant__ G
     }
 }
 
-size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
-
 }  // namespace
 
 // scratch: pair table | row offsets | decisions 4 npairs (G + 1)^2 x 32 bit |

@@ -25,8 +25,6 @@ namespace {
 
 constexpr int64_t kStaticMaxKeypoints = 16384;  // per image (m and n)
 
-constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
-
 // Layout of the scratch array (offsets in bytes).
 constexpr int64_t M = kStaticMaxKeypoints, N = kStaticMaxKeypoints;
 constexpr size_t kOffPairs = 0;
