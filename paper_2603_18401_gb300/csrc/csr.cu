@@ -342,7 +342,10 @@ cudaError_t launch_csr_rows(const Launch &L, int sms, cudaStream_t s) {
     if (L.nq == 0 || L.nr == 0) return cudaSuccess;
     const int words = (int)((std::min<int64_t>(L.max_n, kMaxBits) + 31) / 32);  // the largest image of the call
     const size_t smem = sizeof(uint32_t) * kRowWarps * (size_t)(words + kStage / 2);
-    cudaError_t e = cudaFuncSetAttribute(rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the limit is the function's on the device, shared with other contexts'
+    // threads: always the largest any call needs
+    constexpr int kMostSmem = (int)sizeof(uint32_t) * kRowWarps * (kMaxBits / 32 + kStage / 2);
+    cudaError_t e = cudaFuncSetAttribute(rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rows_kernel, kRowWarps * 32, smem);

@@ -249,7 +249,10 @@ cudaError_t launch_gms(void *scratch, const GmsLayout &l, const GmsPair *one, in
     const int most = std::max((int)(kGmsSmemBudget / column) - 2, 1);
     const int runs = (G1 + most - 1) / most, span = (G1 + runs - 1) / runs;
     const size_t smem = column * (size_t)(span + 2);
-    cudaError_t e = cudaFuncSetAttribute(gms_cells_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the limit is the function's on the device, shared with other contexts'
+    // threads: always the largest any grid needs (the tables of three cells,
+    // the least a block takes, fit the budget up to 48 x 48 cells)
+    cudaError_t e = cudaFuncSetAttribute(gms_cells_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGmsSmemBudget);
     if (e != cudaSuccess) return e;
     const int64_t blocks = std::min<int64_t>((rows + 127) / 128, 152 * 16);
     if ((e = launch_pdl(gms_prep_kernel, dim3((unsigned)blocks), dim3(128), 0, st, a, c1, c2)) != cudaSuccess) return e;
