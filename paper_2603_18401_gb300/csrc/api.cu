@@ -143,6 +143,11 @@ egm_status from_bits(uint32_t st) {
         if (e_ != cudaSuccess) return from_cuda(e_); \
     } while (0)
 
+// Waits for the copies and memsets that the caller issued on the legacy
+// default stream (they may return before the device has done them): a context
+// on a non-blocking stream is not ordered after that stream.
+cudaError_t settle() { return cudaStreamSynchronize(cudaStreamLegacy); }
+
 int row_bytes_of(int kind, int dim) {
     switch (kind) {
         case EGM_DESC_U8_L2: return dim;
@@ -715,6 +720,7 @@ egm_status egm_create(egm_ctx **out, int device, void *stream) {
     if (e == cudaSuccess) e = cudaMallocHost(&c->h_counters, 8 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = grow(c->sc.small, 256);
     if (e == cudaSuccess) e = cudaMemset(c->sc.small.ptr, 0, 256);
+    if (e == cudaSuccess) e = settle();
     if (e != cudaSuccess) {
         egm_destroy(c);
         return from_cuda(e);
@@ -1246,6 +1252,7 @@ egm_status egm_graph_create(egm_ctx *c, const egm_pair *pairs, int32_t npairs, c
     if (e == cudaSuccess)
         e = cudaMemcpy(g->sc.offs.ptr, h.data() + sizeof(PairDesc) * npairs, ob, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(g->sc.small.ptr, 0, 256);
+    if (e == cudaSuccess) e = settle();
     if (e == cudaSuccess && tune) {
         // tune on the graph's own scratch before capturing
         s = tune_regime(c, g->sc, pl, npairs, out, band, shape);
@@ -1349,6 +1356,7 @@ egm_status egm_mlp_create(egm_ctx *c, const float *params, egm_mlp **out) {
     if (e == cudaSuccess) e = cudaMemset(m->v.ptr, 0, pb);
     if (e == cudaSuccess) e = cudaMemset(m->grad.ptr, 0, pb);
     if (e == cudaSuccess) e = cudaMemset(m->loss.ptr, 0, 64);
+    if (e == cudaSuccess) e = settle();
     if (e != cudaSuccess) {
         egm_mlp_destroy(m);
         return from_cuda(e);
@@ -1384,11 +1392,13 @@ egm_status egm_mlp_get_state(egm_mlp *m, float *params, float *am, float *av, in
 egm_status egm_mlp_set_state(egm_mlp *m, const float *params, const float *am, const float *av, int64_t step) {
     if (!m || step < 0) return EGM_ERR_ARG;
     EGM_TRY(cudaSetDevice(m->ctx->device));
-    EGM_TRY(cudaStreamSynchronize(m->ctx->stream));
+    // on the context's stream, between its earlier and later calls
+    cudaStream_t st = m->ctx->stream;
     const size_t pb = sizeof(float) * EGM_MLP_PARAMS;
-    if (params) EGM_TRY(cudaMemcpy(m->params.ptr, params, pb, cudaMemcpyHostToDevice));
-    if (am) EGM_TRY(cudaMemcpy(m->m.ptr, am, pb, cudaMemcpyHostToDevice));
-    if (av) EGM_TRY(cudaMemcpy(m->v.ptr, av, pb, cudaMemcpyHostToDevice));
+    if (params) EGM_TRY(cudaMemcpyAsync(m->params.ptr, params, pb, cudaMemcpyHostToDevice, st));
+    if (am) EGM_TRY(cudaMemcpyAsync(m->m.ptr, am, pb, cudaMemcpyHostToDevice, st));
+    if (av) EGM_TRY(cudaMemcpyAsync(m->v.ptr, av, pb, cudaMemcpyHostToDevice, st));
+    EGM_TRY(cudaStreamSynchronize(st));  // the caller's arrays are read
     m->step = step;
     return EGM_OK;
 }
