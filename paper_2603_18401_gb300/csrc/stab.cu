@@ -606,37 +606,70 @@ constexpr int kChunkQ = 8; // queries per warp whose windows are computed in one
 // of the pair's queries (key_window_span with the pair's extremes of the pad
 // arguments and of |key|, recorded by the prep kernel): a superset of each
 // query's own window, so the exact test keeps the same candidates.
+//
+// Where F has rank 2 to rounding, the lines pass the epipole within far less
+// than a pixel and the extremes add nothing.  Where it has not (an estimate
+// whose rank was not enforced), a line's distance from the epipole grows
+// towards the epipole of image 1, and one query there would widen every
+// window of the pair: levels that the extremes widen by more than about a
+// fourth over the pair's best query take each query's own half-width instead.
+// (16,384 keypoints at 2 px, epipoles inside, the smallest singular value 1e-4
+// of the second: mutual match 308 us against 1,614 with the extremes, 8 pairs 414
+// against 6,329, one u8 pair 250 against 889, one float pair 268 against 1,319.
+// What is left is the query next to the epipole itself, whose window is the
+// image: its warp walks 15,000 references alone, 135 us; without the five
+// keypoints within 30 px the mutual match takes 150.  Loading its records
+// several steps ahead, in a function of its own or into the L1 cache, shortens
+// that walk by a quarter at most and slows every other call.)
+enum : int { kWinShared = 0, kWinWhole = 1, kWinOwn = 2 };
 struct LevelWin {
     float hw;      // half-width of every window in the level's key space
-    int whole;     // 1: every window covers the whole level
+    int kind;      // kWinShared; kWinWhole: every window covers the whole level; kWinOwn: a half-width per query
     uint32_t s, e; // sorted positions of the level
     int sh;        // key bits below the level's buckets
 };
 
 __device__ __forceinline__ LevelWin level_win(const PairGeom &G, int lv) {
-    const float a0 = G.mode == kModeAngular ? __uint_as_float(G.qa0max) : __uint_as_float(G.qa0min);
-    const KeyWin w = key_window_span(G, lv, 0.0f, 0.0f, __uint_as_float(G.qkabs), a0, __uint_as_float(G.qa1max),
-                                     false);
+    const bool angular = G.mode == kModeAngular;
+    const float a0min = __uint_as_float(G.qa0min), a0max = __uint_as_float(G.qa0max), a1max = __uint_as_float(G.qa1max);
+    const KeyWin w = key_window_span(G, lv, 0.0f, 0.0f, __uint_as_float(G.qkabs), angular ? a0max : a0min, a1max, false);
     LevelWin c;
     c.hw = w.hi;
-    c.whole = w.kind == 1 ? 1 : 0;
+    c.kind = w.kind == 1 ? kWinWhole : kWinShared;
+    // the half-width's leading term is (smax dmin + a0) / dmin, or (smax + R a1) / a0 in the parallel frame
+    const float smax = __uint_as_float(G.smax[lv]), dmin = __uint_as_float(G.dmin[lv]), R = __uint_as_float(G.tmax[lv]);
+    if (angular ? smax < 1.0f && a0max > 1.25f * a0min + 0.25f * (smax * dmin)
+                : smax + R * a1max > 1.25f * (a0min * smax))
+        c.kind = kWinOwn;
     c.s = G.start[lv];
     c.e = G.start[lv + 1];
     c.sh = kQBits - G.bits[lv];
     return c;
 }
 
-// The window of query r in the lane's level as bucket-table indices (the
+// The half-width of query r's own window in level lv, infinite where the
+// window is the whole level.
+__device__ __forceinline__ float own_half_width(const PairGeom &G, int lv, const QueryRec &r) {
+    const KeyWin w = key_window_span(G, lv, 0.0f, 0.0f, fabsf(r.key), r.aux0, r.aux1, false);
+    return w.kind == 2 ? w.hi : INFINITY;
+}
+
+// The window of query r in the lane's level lv as bucket-table indices (the
 // kinds of WinKeys).
-__device__ __forceinline__ WinKeys level_window(const PairGeom &G, const LevelWin &c, const QueryRec &r) {
+__device__ __forceinline__ WinKeys level_window(const PairGeom &G, const LevelWin &c, int lv, const QueryRec &r) {
     WinKeys k;
     k.s = c.s;
     k.e = c.e;
     k.ta = k.tb = 0u;
     k.kind = 0;
     if (r.flags & EGM_FLAG_DEGENERATE_LINE) return k;
-    const bool full = c.whole || (r.flags & kQExactOnly) != 0;
-    const float lo = r.key - c.hw, hi = r.key + c.hw;
+    bool full = c.kind == kWinWhole || (r.flags & kQExactOnly) != 0;
+    float hw = c.hw;
+    if (c.kind == kWinOwn && !full) {
+        hw = own_half_width(G, lv, r);
+        full = !(hw < INFINITY);
+    }
+    const float lo = r.key - hw, hi = r.key + hw;
     const bool low = G.mode == kModeAngular && lo < -kHalfPiF;
     const bool high = G.mode == kModeAngular && hi >= kHalfPiF;
     if (full || (low && high)) {
@@ -749,7 +782,7 @@ __global__ void __launch_bounds__(kPairThreads, KIND == EGM_DESC_F32_L2 ? 8 : ON
         const int sl = s0 + lane;
         if (sl < nk * nlev) {
             const int k = sl / nlev, l = sl - k * nlev;
-            const WinKeys wk = level_window(W.g, W.win[l], qchunk[warp][k]);
+            const WinKeys wk = level_window(W.g, W.win[l], W.lv[l], qchunk[warp][k]);
             uint32_t a = 0, b = 0;
             if (wk.kind >= 2) {
                 const uint32_t *Tl = L.tab + PD.t_off + W.g.tab[W.lv[l]];
