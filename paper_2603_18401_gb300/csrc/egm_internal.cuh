@@ -640,7 +640,8 @@ struct GmsPair {
     double w1, h1, w2, h2;
 };
 struct GmsLayout {
-    size_t table, offs, dec, c1, c2, total;
+    size_t table, offs, dec, c1, c2, ds, total;
+    bool sorted;  // the matches are sorted by cell first (ds)
 };
 GmsLayout gms_layout(int npairs, int64_t rows, int grid);
 // several pairs: the pair table and row offsets are already in the scratch at
