@@ -97,7 +97,9 @@ constexpr int kRowWarps = 4;
 constexpr int kShortRow = 64;             // longest row sorted in registers
 constexpr int kStage = 768;              // row entries (16-bit, from the step's first) staged for coalesced stores
 constexpr uint32_t kLaneWords = 31;       // most bitmap words a lane walks per step; odd, and 32 * 32 * 31 < 2^16
-constexpr int kMaxBits = 1 << 18;         // bitmap bits per warp: longer index ranges take several passes
+constexpr int kMaxBits = 1 << 16;         // bitmap bits per warp: longer index ranges take several passes
+constexpr int kSortRow = 1024;            // longest row sorted in registers there
+static_assert(kSortRow <= kMaxBits / 32, "the bitmap's memory holds the row's candidates");
 
 // Ascending sort of K = 32 or 64 keys, one or two per lane (lane l holds keys
 // l and 32 + l), by a bitonic network: the step across 32 keys pairs the
@@ -128,6 +130,58 @@ __device__ __forceinline__ void sort_lanes(uint32_t &a, uint32_t &b, int lane) {
     }
 }
 
+// Ascending sort of K = 128 to 1024 keys, K / 32 per lane (lane l holds
+// keys l, l + 32, ...), by a bitonic network: steps across 32 keys and more pair
+// a lane's own keys, the others are shuffles.  (The loops over the shuffles'
+// distances are not unrolled: of 512 keys 550 instructions in the place of
+// 2,900.)
+template <int K>
+__device__ __forceinline__ void sort_regs(uint32_t (&a)[K / 32], int lane) {
+    constexpr int R = K / 32;
+    auto across = [&](int j, int r, bool up) {
+        const uint32_t o = __shfl_xor_sync(0xffffffffu, a[r], j);
+        a[r] = ((lane & j) == 0) == up ? min(a[r], o) : max(a[r], o);
+    };
+#pragma unroll 1
+    for (int k = 2; k <= 16; k <<= 1)
+#pragma unroll 1
+        for (int j = k >> 1; j > 0; j >>= 1)
+#pragma unroll
+            for (int r = 0; r < R; r++) across(j, r, (lane & k) == 0);
+#pragma unroll
+    for (int q = 1; q <= R; q <<= 1) {  // blocks of 32 q keys
+#pragma unroll
+        for (int h = q >> 1; h > 0; h >>= 1)
+#pragma unroll
+            for (int r = 0; r < R; r++)
+                if ((r & h) == 0) {
+                    const bool up = q == R || (r & q) == 0;
+                    const uint32_t lo = min(a[r], a[r | h]), hi = max(a[r], a[r | h]);
+                    a[r] = up ? lo : hi;
+                    a[r | h] = up ? hi : lo;
+                }
+#pragma unroll 1
+        for (int j = 16; j > 0; j >>= 1)
+#pragma unroll
+            for (int r = 0; r < R; r++) across(j, r, q == R || (r & q) == 0);
+    }
+}
+
+// `have` <= K keys of `list` in ascending order to `out`; the list is zero afterwards.
+template <int K>
+__device__ __forceinline__ void write_sorted(uint32_t *list, uint32_t have, int32_t *out, int lane) {
+    uint32_t a[K / 32];
+#pragma unroll
+    for (int r = 0; r < K / 32; r++) {
+        a[r] = (uint32_t)(32 * r + lane) < have ? list[32 * r + lane] : ~0u;
+        list[32 * r + lane] = 0u;
+    }
+    sort_regs<K>(a, lane);
+#pragma unroll
+    for (int r = 0; r < K / 32; r++)
+        if ((uint32_t)(32 * r + lane) < have) out[32 * r + lane] = (int32_t)a[r];
+}
+
 // One warp per query.  The query's windows are computed by its lanes (lane =
 // level) and flattened by a prefix sum; the warp tests 32 window elements per
 // step.  Rows of up to 64 candidates are collected and sorted in registers.
@@ -149,8 +203,16 @@ __device__ __forceinline__ void sort_lanes(uint32_t &a, uint32_t &b, int lane) {
 // 15 words: 10 % more time on the whole call than 31).  The staging buffer is
 // 16-bit and no larger than 28 resident warps per SM allow, which is also the
 // registers' limit (1024 entries: 24 warps, 4 % on the whole call).
-// Index ranges beyond kMaxBits take one pass over the windows per range.
-__global__ void __launch_bounds__(kRowWarps * 32) rows_kernel(Launch L, int words) {
+//
+// Index ranges beyond kMaxBits take one pass over the windows per range, and
+// medium rows there are collected and sorted in registers (LARGE: an instance
+// of its own, for calls with such an image).  With one bitmap for up to 262,144
+// references, whose memory left one block per SM, and every row walked from it:
+// offsets and rows of 20,000 queries of 100 candidates each 429 us at 262,144
+// references and 1,870 at 1,048,576, now 65 and 112; of 500 candidates 630 and
+// 2,330, now 200 and 253.
+template <bool LARGE>
+__global__ void __launch_bounds__(kRowWarps * 32, LARGE ? 5 : 0) rows_kernel(Launch L, int words) {
     pdl_begin();
     extern __shared__ __align__(16) uint32_t rsm[];
     if (L.cand_offsets[L.nq] > L.cand_capacity) return;  // capacity error: no row is written
@@ -266,6 +328,25 @@ __global__ void __launch_bounds__(kRowWarps * 32) rows_kernel(Launch L, int word
             __syncwarp();
             continue;
         }
+        // sorted in registers; of two ranges (two passes) rows of up to 512 only: up to 1024, 189 us against 175 with the
+        // passes (131,072 references, rows of about 500), of four ranges 198 against 285
+        if (LARGE && n > (uint32_t)kMaxBits && len <= (n > 2u * kMaxBits ? (uint32_t)kSortRow : kSortRow / 2u)) {
+            uint32_t count = 0;  // the candidates, in the bitmap's memory
+            visit([&](bool cand, uint32_t j) {
+                const uint32_t m = __ballot_sync(0xffffffffu, cand);
+                const uint32_t slot = count + (uint32_t)__popc(m & lt);
+                if (cand && slot < len) bm[slot] = j;
+                count += (uint32_t)__popc(m);
+            });
+            __syncwarp();
+            const uint32_t have = min(count, len);
+            if (have <= 128u) write_sorted<128>(bm, have, out, lane);
+            else if (have <= 256u) write_sorted<256>(bm, have, out, lane);
+            else if (have <= 512u) write_sorted<512>(bm, have, out, lane);
+            else write_sorted<kSortRow>(bm, have, out, lane);
+            __syncwarp();
+            continue;
+        }
         const uint32_t nbits = 32u * (uint32_t)words;
         uint32_t done = 0;  // entries of the row written
         for (uint32_t j0 = 0; j0 < n; j0 += nbits) {
@@ -341,17 +422,19 @@ cudaError_t launch_csr_offsets(const Launch &L, cudaStream_t s) {
 cudaError_t launch_csr_rows(const Launch &L, int sms, cudaStream_t s) {
     if (L.nq == 0 || L.nr == 0) return cudaSuccess;
     const int words = (int)((std::min<int64_t>(L.max_n, kMaxBits) + 31) / 32);  // the largest image of the call
+    const bool large = L.max_n > kMaxBits;
+    const auto kernel = large ? rows_kernel<true> : rows_kernel<false>;
     const size_t smem = sizeof(uint32_t) * kRowWarps * (size_t)(words + kStage / 2);
     // the limit is the function's on the device, shared with other contexts'
     // threads: always the largest any call needs
     constexpr int kMostSmem = (int)sizeof(uint32_t) * kRowWarps * (kMaxBits / 32 + kStage / 2);
-    cudaError_t e = cudaFuncSetAttribute(rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rows_kernel, kRowWarps * 32, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kRowWarps * 32, smem);
     if (e != cudaSuccess) return e;
     const int64_t blocks = std::min<int64_t>((L.nq + kRowWarps - 1) / kRowWarps, (int64_t)std::max(per_sm, 1) * sms);
-    return launch_pdl(rows_kernel, dim3((unsigned)blocks), dim3(kRowWarps * 32), smem, s, L, words);
+    return launch_pdl(kernel, dim3((unsigned)blocks), dim3(kRowWarps * 32), smem, s, L, words);
 }
 
 }  // namespace egm
