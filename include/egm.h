@@ -150,7 +150,10 @@ enum {
                               128-query tiles per SM, or when every pair has u8
                               descriptors, a scalar eps and an expected 32 or more
                               candidates per query (2 eps n / (W H) x 0.8 of the
-                              image diagonal); plain otherwise */
+                              image diagonal); plain otherwise.  With candidate
+                              lists: such dense pairs of at most twice as many
+                              references as queries, and other calls whose expected
+                              candidates and queries outweigh their references */
     EGM_FORM_PLAIN = 1,    /* windowed stabbing + CUDA-core descriptor distances */
     EGM_FORM_BANDED = 2    /* angle-banded tiles, descriptor dot products on tensor cores */
 };

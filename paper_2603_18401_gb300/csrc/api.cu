@@ -284,17 +284,50 @@ size_t offs_entries(int npairs, int64_t nq) {
     return 3 * (size_t)(npairs + 1) + (size_t)(nq / band_tile_queries() + npairs + 2) + 1;
 }
 
+// What the banded form saves on a call with candidate lists, in us: only the
+// counts and the best two come from it, its rows are written by the same kernel,
+// so it pays later than without lists.  Per query, expected candidate and
+// reference, less a constant (the side stream's fork and join, the queries'
+// order, a band tile's set-up); fitted to 572 calls of one pair (2,000 to 120,000
+// queries, 2,000 to 200,000 references, 4 to 1,200 candidates a query) and of 2
+// to 256, both forms measured: the form it picks takes 0.2 % longer than the
+// better one on average for u8 and binary rows, 0.7 % for float rows, 9 % at
+// most (float rows 18 %).  50,000 x 50,000 keypoints: 20 candidates 194 us plain, 227
+// banded; 160: 324 and 300; 1,200: 997 and 547.  50,000 x 200,000: 20: 273 and 419.
+double list_gain(const Plan &pl) {
+    struct Fit {
+        double query, cand, ref, fixed;
+    };
+    static const Fit u8{3.1e-4, 8.0e-6, 2.9e-4, 38.0}, bin{5.4e-4, 4.0e-6, 2.4e-4, 57.0},
+        f32{8.4e-4, 1.02e-5, 7.4e-4, 69.0}, mixed{1.6e-3, 8.0e-5, 1.6e-3, 52.0};  // (mixed: a slower plain kernel)
+    const Fit &f = pl.kinds == 1u << EGM_DESC_U8_L2    ? u8
+                   : pl.kinds == 1u << EGM_DESC_BIN    ? bin
+                   : pl.kinds == 1u << EGM_DESC_F32_L2 ? f32
+                                                       : mixed;
+    // with tolerances per keypoint the density is not known here: 48 candidates a query
+    const double cand = pl.eps_vec ? 48.0 * (double)pl.nq : pl.kbar_q;
+    return f.query * (double)pl.nq + f.cand * cand - f.ref * (double)pl.nr - f.fixed;
+}
+
 // The banded form runs when every pair fits it and it is requested (without
 // candidate lists) -- or left to the library and either the call has
 // more than two tiles per SM or its u8 pairs are dense (about 32 or more
-// candidates per query).  With few tiles of sparse pairs every CTA of the
+// candidates per query).  With candidate lists: dense u8 pairs as well, where
+// the references are at most twice the queries (the documented choice, though
+// the plain form lists up to about 160 candidates a query sooner: 8,000 x 8,000
+// keypoints, 40 candidates 114 us against 159), and else when it saves time
+// (list_gain): with more references each tile's band is long for what its queries
+// find, with many tiles of sparse pairs the plain form's one pass is short.
+// With few tiles of sparse pairs every CTA of the
 // band kernel takes one latency-bound tile and the plain form (no query
 // sort, no packing) finishes first; with many tiles the banded form's
 // throughput wins, and on dense pairs its tensor-core distances beat one
 // CUDA-core distance per candidate.
 egm_status choose_band(const Plan &pl, const egm_params &prm, bool csr, int sms, bool &band) {
     band = pl.band_ok && ((prm.form == EGM_FORM_BANDED && !csr) ||
-                          (prm.form == EGM_FORM_AUTO && (pl.ntiles > 2 * (int64_t)sms || pl.dense_u8)));
+                          (prm.form == EGM_FORM_AUTO &&
+                           ((pl.dense_u8 && !(csr && pl.nr > 2 * pl.nq)) ||
+                            (csr ? list_gain(pl) > 0.0 : pl.ntiles > 2 * (int64_t)sms))));
     if (prm.form == EGM_FORM_BANDED && !band) return EGM_ERR_UNIMPLEMENTED;
     return EGM_OK;
 }
