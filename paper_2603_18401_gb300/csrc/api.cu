@@ -627,11 +627,14 @@ cudaError_t time_config(egm_ctx *c, Scratch &sc, const Plan &pl, int npairs, con
 // The configuration of a call.  Forced choices (plain form, a forced shape)
 // need no timing; with candidate lists or params.tune == 0 the heuristic of
 // choose_band picks the form, and the shape is (1 box, 4 CTAs per SM), but on
-// dense u8 pairs of more than 8/3 tiles per SM, whose tiles are not split any
-// more there, (4 boxes, 2 CTAs).  (50,000 keypoints at 50 px, 2.6 tiles per SM:
-// 223 us a call against 250; 30,000 at 20 px 113 against 134; 70,000 at 20 px, 3.6
-// tiles per SM: 257 against 218.)  Otherwise the regime's entry
-// in the tuner's cache decides, and `tune` asks the caller to time the
+// dense u8 pairs of more than 10/3 tiles per SM (4 boxes, 2 CTAs): there a
+// tile is one or two items in either shape, below it three and more fill the
+// four CTAs.  (Calls at 20 and 50 px, the first shape against the second:
+// 50,000 keypoints, 2.6 tiles per SM, 164 against 211 us and 238 against 262;
+// 54,000 182 against 196 and 236 against 268; 62,000, 3.2 per SM, 241 against
+// 243 and 289 against 325; 66,000, 3.4 per SM, 268 against 231 and 437 against
+// 379; 76,000 295 against 243 and 492 against 386.)  Otherwise the regime's
+// entry in the tuner's cache decides, and `tune` asks the caller to time the
 // candidates first (the regime has none yet).
 egm_status choose_config(const egm_ctx *c, const Plan &pl, int npairs, bool csr, bool &band, int &shape,
                          bool &tune) {
@@ -646,7 +649,7 @@ egm_status choose_config(const egm_ctx *c, const Plan &pl, int npairs, bool csr,
         egm_status s = choose_band(pl, prm, csr, c->sms, band);
         if (s != EGM_OK) return s;
         // many tiles of wide bands (dense pairs): fewer, larger chunks
-        shape = forced >= 0 ? forced : pl.dense_u8 && 3 * pl.ntiles > 8 * (int64_t)c->sms ? 0 : 2;
+        shape = forced >= 0 ? forced : pl.dense_u8 && 3 * pl.ntiles > 10 * (int64_t)c->sms ? 0 : 2;
         return EGM_OK;
     }
     const auto it = c->tuned.find(regime_key(pl, npairs));
