@@ -133,8 +133,8 @@ __device__ __forceinline__ void copy16(void *dst, const void *src, int bytes, in
 }
 
 // Matching (match: some pair has descriptors) and, when L.qcount is set, the
-// candidates per query.  (A single pair with u8 or binary rows runs
-// stab_pair_kernel instead.)
+// candidates per query.  (Rows of the usual kinds and sizes run
+// stab_pair_kernel instead, see launch_warp_per_query.)
 template <int KIND>
 __global__ void __launch_bounds__(kStabThreads, 4) stab_kernel(Launch L) {
     pdl_begin();
@@ -378,8 +378,9 @@ __global__ void __launch_bounds__(kStabThreads, 4) stab_kernel(Launch L) {
                             nexact++;
                         }
                     }
-                    if (cand) atomicAdd(&S.cnt[qq], 1u);
-                    if (match) {
+                    if (!match) {
+                        if (cand) atomicAdd(&S.cnt[qq], 1u);
+                    } else {
                         // warp-aggregated append to the round's candidate list
                         const uint32_t m = __ballot_sync(0xffffffffu, cand);
                         if (m) {
@@ -399,6 +400,8 @@ __global__ void __launch_bounds__(kStabThreads, 4) stab_kernel(Launch L) {
             }
             __syncthreads();
             const uint32_t nc = S.ncand;
+            // the round's candidates per query (rather than one more atomic add per candidate)
+            if (match && tid < kQB) S.cnt[tid] += S.rcnt[tid];
             if (match && nc > 0) {
                 // 2a': segments by query
                 if (warp == 0) {
