@@ -25,18 +25,16 @@ namespace {
 
 constexpr int64_t kStaticMaxKeypoints = 16384;  // per image (m and n)
 
-// Layout of the scratch array (offsets in bytes).
+// Layout of the scratch array (offsets in bytes).  Its pairs always take
+// build_kernel, which needs no keys, unsorted records or cursors in memory.
 constexpr int64_t M = kStaticMaxKeypoints, N = kStaticMaxKeypoints;
 constexpr size_t kOffPairs = 0;
 constexpr size_t kOffGeom = align256(kOffPairs + sizeof(PairDesc));
 constexpr size_t kOffOffs = align256(kOffGeom + sizeof(PairGeom));
-constexpr size_t kOffKeys = align256(kOffOffs + 4 * sizeof(int64_t));
-constexpr size_t kOffRec = align256(kOffKeys + sizeof(uint32_t) * N);
-constexpr size_t kOffRtmp = align256(kOffRec + sizeof(float4) * N);
-constexpr size_t kOffTab = align256(kOffRtmp + sizeof(float4) * N);
+constexpr size_t kOffRec = align256(kOffOffs + 4 * sizeof(int64_t));
+constexpr size_t kOffTab = align256(kOffRec + sizeof(float4) * N);
 constexpr int64_t kTabCap = 4 * N + 2 * kLevels + 32;
-constexpr size_t kOffCurs = align256(kOffTab + sizeof(uint32_t) * kTabCap);
-constexpr size_t kOffQrec = align256(kOffCurs + sizeof(uint32_t) * kTabCap);
+constexpr size_t kOffQrec = align256(kOffTab + sizeof(uint32_t) * kTabCap);
 constexpr size_t kOffQcount = align256(kOffQrec + sizeof(QueryRec) * M);
 constexpr size_t kOffScan = align256(kOffQcount + sizeof(uint32_t) * (M + 4));
 constexpr size_t kOffBlk = align256(kOffScan + sizeof(int64_t) * (M / kCountTile + 2));
@@ -158,12 +156,9 @@ extern "C" egm_status egm_match_pair_static(const egm_pair *P, const egm_out *ou
     L.nr = P->n;
     L.q_offs = reinterpret_cast<const int64_t *>(base + kOffOffs);
     L.r_offs = reinterpret_cast<const int64_t *>(base + kOffOffs) + 2;
-    L.key_a = reinterpret_cast<uint32_t *>(base + kOffKeys);
     L.rec = reinterpret_cast<float4 *>(base + kOffRec);
-    L.rtmp = reinterpret_cast<float4 *>(base + kOffRtmp);
     L.tab = reinterpret_cast<uint32_t *>(base + kOffTab);
     L.ntab = pd.t_cap;
-    L.curs = reinterpret_cast<uint32_t *>(base + kOffCurs);
     L.prep_done = reinterpret_cast<uint32_t *>(base + kOffSmall) + 40;
     L.qrec = reinterpret_cast<QueryRec *>(base + kOffQrec);
     L.status = reinterpret_cast<uint32_t *>(base + kOffSmall);
