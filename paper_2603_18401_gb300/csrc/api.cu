@@ -82,7 +82,7 @@ struct egm_ctx {
     DevBuf stage;  // host-path staging of inputs and outputs
     DevBuf compact;  // tile counts of egm_compact_matches
     DevBuf ft;       // egm_match_mutual_pair: F^T of the reverse direction
-    DevBuf gms;      // egm_gms: pair table, matches sorted by cell, decisions per grid shift
+    DevBuf gms;      // egm_gms: pair table, cells of the matches (and their sorted lists), decisions per grid shift
     void *gms_host = nullptr;        // pinned staging of the GMS pair table
     size_t gms_host_bytes = 0;
     cudaEvent_t gms_host_ev = nullptr;
@@ -555,7 +555,9 @@ cudaError_t enqueue_pipeline(const Launch &L, Scratch &sc, bool csr, int max_n, 
     if (band) EGM_Q(launch_pack(L, st));  // float pairs only
     if (tc) EGM_Q(mark(tc, tb, 4));
     if (band) {
-        // a tile that gives up (EGM_ERR_TIMEOUT) leaves its counts at zero
+        // tiles that a CTA never starts after a wait gave up (EGM_ERR_TIMEOUT) leave their counts at
+        // zero, the tile it gave up in those of its tested chunks: such rows are cut short, and the row
+        // writer writes no more entries than a query's count
         if (csr) EGM_Q(cudaMemsetAsync(L.qcount, 0, sizeof(uint32_t) * (size_t)L.nq, st));
         if (shape >= 0) EGM_Q(launch_band(L, sms, shape, st, false));
     } else {

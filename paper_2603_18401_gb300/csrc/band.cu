@@ -661,7 +661,7 @@ __device__ __forceinline__ uint32_t sw128(int r, int c) { return (uint32_t)(r * 
 // number g of the CTA:
 //   records, u8 norms, binary rows   kRS slots (g mod kRS); a slot is reused
 //                                    once the consumers have finished its chunk
-//   operand stages                   2 (g mod 2); reused once the chunk's MMA is done
+//   operand stages                   kNB, two or three (g mod kNB); reused once the chunk's MMA is done
 //   accumulators                     kNA (g mod kNA); reused once the consumers
 //                                    have read them
 // so the producer runs up to kNA - 1 chunks ahead of the consumers and the
@@ -994,8 +994,8 @@ __global__ void __launch_bounds__(kBandThreads, CPS)
                     if (flt) tc::bulk_load(&S.u.io.rn[FLT ? s : 0][bb][0], L.rnorm + row, kBoxR * 16, &S.fullR[s]);
                 }
             };
-            // float rows of chunk c by TMA into operand stage g mod 2, once the
-            // MMA of chunk g - 2 is done (control thread)
+            // float rows of chunk c by TMA into operand stage g mod kNB, once the
+            // MMA of chunk g - kNB is done (control thread)
             auto issueB = [&](int c) {
                 const uint32_t g = seq + (uint32_t)c, st = g % kNB;
                 if (g >= (uint32_t)kNB && !wait(&S.sfree[st], ((g - kNB) / kNB) & 1u)) return;
@@ -1013,7 +1013,7 @@ __global__ void __launch_bounds__(kBandThreads, CPS)
             };
             // u8 and binary rows of chunk c, one row per lane and box, by the
             // indices in its records: u8 bytes into K half 1 of operand stage
-            // g mod 2 (128-byte swizzle), once the MMA of chunk g - 2 is done;
+            // g mod kNB (128-byte swizzle), once the MMA of chunk g - kNB is done;
             // binary rows into slot g mod kRS of B[0][0] (free: its records'
             // slot was).  Returns the boxes whose row this lane copied.
             // Records are copied in chunk order as far ahead as their slots allow,

@@ -671,11 +671,11 @@ int mlp_param_count();
 // gradient and loss added to grad and loss; a timed-out MMA wait sets kStTimeout in *err
 cudaError_t launch_mlp_train(const float *params, const float *feat, const float *resid, int64_t n, float q,
                              float *grad, float *loss, uint32_t *err, int sms, cudaStream_t s);
-// one Adam step; clears grad and loss, the loss going to `out` first (device, may be NULL)
 // The gradient and the loss into the caller's buffers (each may be null) and
 // *err into *host_err (pinned); all three are zero again afterwards.
 cudaError_t launch_hand_out(float *g, float *loss, uint32_t *err, float *gout, float *lout, uint32_t *host_err,
                             cudaStream_t s);
+// one Adam step; clears grad and loss, the loss going to `out` first (device, may be NULL)
 cudaError_t launch_adam(float *p, float *g, float *m, float *v, float lr, int64_t step, float *loss, float *out,
                         cudaStream_t s);
 cudaError_t launch_residuals(const double *xy1, const double *xy2, const double *F, int64_t m, int64_t n,

@@ -175,30 +175,28 @@ __device__ __forceinline__ QueryRec prep_query(const Launch &L, const PairView &
 }
 
 // The extremes over a pair's queries of what their windows are padded by, from
-// a converged warp's records (valid: the lane has one); the single-pair
-// stabbing kernel's per-level windows cover every query with them.
+// a converged warp's records (valid: the lane has one), warp-aggregated; the
+// warp-per-query matching kernel's per-level windows cover every query with them.
 __device__ __forceinline__ void query_extremes(const Launch &L, bool valid, int p, const QueryRec &r) {
     const int lane = threadIdx.x & 31;
     const bool use = valid && r.flags == 0u;
     const uint32_t qgroup = use ? (uint32_t)p : 0xffffffffu;
     const uint32_t qa0 = use ? __float_as_uint(r.aux0) : 0u, qa1 = use ? __float_as_uint(r.aux1) : 0u;
     const uint32_t qk = use ? __float_as_uint(fabsf(r.key)) : 0u;
-// warp-aggregated query extremes of each pair (the single-pair
-// stabbing kernel's per-level windows cover every query with them)
-if (__any_sync(0xffffffffu, qgroup != 0xffffffffu)) {
-    const uint32_t qpeers = __match_any_sync(0xffffffffu, qgroup);
-    const uint32_t a0x = __reduce_max_sync(qpeers, qa0);
-    const uint32_t a0n = __reduce_min_sync(qpeers, qgroup == 0xffffffffu ? 0x7f800000u : qa0);
-    const uint32_t a1x = __reduce_max_sync(qpeers, qa1);
-    const uint32_t kx = __reduce_max_sync(qpeers, qk);
-    if (qgroup != 0xffffffffu && lane == __ffs(qpeers) - 1) {
-        PairGeom &G = L.geom[qgroup];
-        atomicMax(&G.qa0max, a0x);
-        atomicMin(&G.qa0min, a0n);
-        atomicMax(&G.qa1max, a1x);
-        atomicMax(&G.qkabs, kx);
+    if (__any_sync(0xffffffffu, qgroup != 0xffffffffu)) {
+        const uint32_t qpeers = __match_any_sync(0xffffffffu, qgroup);
+        const uint32_t a0x = __reduce_max_sync(qpeers, qa0);
+        const uint32_t a0n = __reduce_min_sync(qpeers, qgroup == 0xffffffffu ? 0x7f800000u : qa0);
+        const uint32_t a1x = __reduce_max_sync(qpeers, qa1);
+        const uint32_t kx = __reduce_max_sync(qpeers, qk);
+        if (qgroup != 0xffffffffu && lane == __ffs(qpeers) - 1) {
+            PairGeom &G = L.geom[qgroup];
+            atomicMax(&G.qa0max, a0x);
+            atomicMin(&G.qa0min, a0n);
+            atomicMax(&G.qa1max, a1x);
+            atomicMax(&G.qkabs, kx);
+        }
     }
-}
 }
 
 }  // namespace

@@ -735,9 +735,10 @@ __device__ __forceinline__ int load_pair_work(PairWork &W, const PairGeom *src, 
 // queries in turn and, within a run, the queries of one pair at a time: its
 // own copy of the pair's geometry, so that no block-wide phase exists either.
 // (Two directions of a 16,384-keypoint pair, tolerances per keypoint: 112 us
-// in blocks of 32 queries, 48 us here; one float pair of 16,384
-// keypoints at 2 px 86 -> 48 us a call, at 8 px 279 -> 74.)  Blocks per SM: 13 for one pair (12: 1 % slower over nine pairs, 16: 2
-// %), 16 for several (13: 4 % slower), 8 for float rows (128 registers).
+// in blocks of 32 queries, 48 us here; one float pair of 16,384 keypoints at
+// 2 px 86 -> 48 us a call, at 8 px 279 -> 74.)  Blocks per SM: 13 for one pair
+// (12: 1 % slower over nine pairs, 16: 2 %), 16 for several (13: 4 % slower),
+// 8 for float rows (128 registers).
 template <int KIND, int G, int C, bool ONE>
 __global__ void __launch_bounds__(kPairThreads, KIND == EGM_DESC_F32_L2 ? 8 : ONE ? 13 : 16)
     stab_pair_kernel(const __grid_constant__ Launch L, int64_t run) {
