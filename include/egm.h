@@ -444,7 +444,8 @@ egm_status egm_mlp_set_fallback(egm_mlp *mlp, double eps_px);
  * features) enter as the sum of two BF16 parts, about 2^-17 relative each, and
  * are summed in FP32 within 128 samples before FP32 sums take over; against
  * FP64 the gradient is no further off than with FP32 operands (relative, in
- * the 2-norm: 1.3e-7 to 2.2e-7 at 1,000 to 65,536 samples, 1.5e-7 to 3.6e-7).  EGM_ERR_TIMEOUT if a tensor-core wait
+ * the 2-norm: 1.1e-7 to 2.2e-7 at 1,000 to 65,536 samples, before 1.5e-7 to
+ * 3.6e-7).  EGM_ERR_TIMEOUT if a tensor-core wait
  * gave up in this call or in an egm_mlp_train_step since the last report (the
  * gradients concerned are not usable); egm_mlp_get_state reports it too. */
 egm_status egm_mlp_grad(egm_mlp *mlp, const float *feat, const float *resid, int64_t n, float quantile, float *grad,
