@@ -362,6 +362,12 @@ T *half_of(DevBuf &b, int parity) {
     return reinterpret_cast<T *>(static_cast<char *>(b.ptr) + (parity ? (b.bytes / 2) & ~(size_t)255 : 0));
 }
 
+// The boxes of a tile of the call in units of its set-up: a tile of 48 expected
+// candidates a query costs about twice its set-up (see band_split).
+float tile_work(const Plan &pl) {
+    return pl.eps_vec ? 1.0f : (float)(pl.kbar_q / (48.0 * (double)std::max<int64_t>(pl.nq, 1)));
+}
+
 Launch make_launch(Scratch &sc, bool counters_on, const egm_params &prm, const Plan &pl, int npairs,
                    const egm_out *out, bool band = false) {
     Scratch *c = &sc;
@@ -423,8 +429,7 @@ Launch make_launch(Scratch &sc, bool counters_on, const egm_params &prm, const P
         L.arrived = reinterpret_cast<uint32_t *>(b + bl.arrived);
         L.part_items = bl.items;
         L.split = 1;  // the launcher's choice, but for float calls
-        // a tile of 48 expected candidates a query costs about twice its set-up (see band_split)
-        L.tile_work = pl.eps_vec ? 1.0f : (float)(pl.kbar_q / (48.0 * (double)std::max<int64_t>(pl.nq, 1)));
+        L.tile_work = tile_work(pl);
     }
     L.kind = pl.pd.empty() ? -1 : pl.pd[0].kind;
     L.row_bytes = pl.pd.empty() ? -1 : pl.pd[0].row_bytes;
@@ -626,16 +631,33 @@ cudaError_t time_config(egm_ctx *c, Scratch &sc, const Plan &pl, int npairs, con
     return e;
 }
 
+// The tile shape where none is timed: 0 (4 boxes, 2 CTAs per SM) or 2 (1 box, 4
+// CTAs).  Tiles of few boxes spend their time on set-up, which two CTAs per SM
+// share with less contention; tiles of many boxes are split into items, which
+// fill four.  Band stage of one u8 pair of n x n, shape 0 against 2 (us) at 3, 75,
+// 300 and 1,200 candidates a query:
+//   16,384 (0.8 tiles per SM)   22  26    28  35    43  53    92  91
+//   25,000 (1.3)                37  45    50  50    76  62   175 122
+//   38,000 (2.0)                40  47    55  59    82  78   175 158
+//   50,000 (2.6)                45  54    59  70    88  82   185 155
+//   62,000 (3.2)                52  61    71  82   104 124   228 200
+//   70,000 (3.6)                54  64    73  85   107 127     -   -
+//   100,000 (5.1)               91  83   115 107   159 159     -   -
+// So up to 6/5 tiles per SM shape 2 needs 768 candidates a query (16 units of
+// work), up to 8/3 it needs 192 (at 144 shape 0 measures 69 against 72 at 50,000,
+// 60 against 58 for eight pairs of 4,000), from there to four, where shape 0 ends
+// in two full rounds, it does not pay but for the densest, and past four always.
+// (Binary pairs of 192 and more gain as much or more: 25,000 at 300 from 128 to 77.)
+int fixed_shape(const Plan &pl, int sms) {
+    const float work = tile_work(pl);
+    if (5 * pl.ntiles <= 6 * (int64_t)sms) return work >= 16.0f ? 2 : 0;
+    if (3 * pl.ntiles <= 8 * (int64_t)sms) return work >= 4.0f ? 2 : 0;
+    return pl.ntiles <= 4 * (int64_t)sms ? 0 : 2;
+}
+
 // The configuration of a call.  Forced choices (plain form, a forced shape)
 // need no timing; with candidate lists or params.tune == 0 the heuristic of
-// choose_band picks the form, and the shape is (1 box, 4 CTAs per SM), but on
-// dense u8 pairs of more than 10/3 tiles per SM (4 boxes, 2 CTAs): there a
-// tile is one or two items in either shape, below it three and more fill the
-// four CTAs.  (Calls at 20 and 50 px, the first shape against the second:
-// 50,000 keypoints, 2.6 tiles per SM, 164 against 211 us and 238 against 262;
-// 54,000 182 against 196 and 236 against 268; 62,000, 3.2 per SM, 241 against
-// 243 and 289 against 325; 66,000, 3.4 per SM, 268 against 231 and 437 against
-// 379; 76,000 295 against 243 and 492 against 386.)  Otherwise the regime's
+// choose_band picks the form and fixed_shape the shape.  Otherwise the regime's
 // entry in the tuner's cache decides, and `tune` asks the caller to time the
 // candidates first (the regime has none yet).
 egm_status choose_config(const egm_ctx *c, const Plan &pl, int npairs, bool csr, bool &band, int &shape,
@@ -650,8 +672,7 @@ egm_status choose_config(const egm_ctx *c, const Plan &pl, int npairs, bool csr,
     if (!prm.tune || csr) {
         egm_status s = choose_band(pl, prm, csr, c->sms, band);
         if (s != EGM_OK) return s;
-        // many tiles of wide bands (dense pairs): fewer, larger chunks
-        shape = forced >= 0 ? forced : pl.dense_u8 && 3 * pl.ntiles > 10 * (int64_t)c->sms ? 0 : 2;
+        shape = forced >= 0 ? forced : fixed_shape(pl, c->sms);
         return EGM_OK;
     }
     const auto it = c->tuned.find(regime_key(pl, npairs));

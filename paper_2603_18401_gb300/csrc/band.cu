@@ -1731,22 +1731,28 @@ cudaError_t launch_pack(const Launch &L, cudaStream_t s) {
 
 // Items a tile of the call is handed out as: the number that takes least time
 // if an item costs one unit to set up and its share of L.tile_work units of
-// boxes, in as many rounds of CTAs as the items need.  Unsplit, the 391 tiles
-// of 50,000 queries take two rounds of two CTAs per SM, the second three
-// quarters empty, 192 us for the kernel at 1,200 candidates a query; in three
-// items a tile four CTAs per SM take 161.  (Whole calls of one pair, without and
-// with: 50,000 queries 255 and 216 us, 25,000 160 and 122, 30,000 126 and 109, 16,384
-// unchanged at one item a tile; always three rounds of items: 16,384 102 us, 50,000
-// 213.)  The unit: split tiles of 50,000 queries lose 4 % at 55 to 74 candidates a
-// query, are even at 109 to 147, and win from there; tiles that only fill idle
-// CTAs win at 28 (25,000 queries: 98 and 91 us).  At 1,200 candidates a fourth
-// to the whole of the unit's estimate measure within 2 %.
-int band_split(const Launch &L, int64_t slots) {
-    if (L.ntiles >= 4 * slots) return 1;
+// boxes, in as many rounds of CTAs as the items need; a split costs 0.6 of a unit
+// for the merge, and with more items than SMs, where CTAs share an SM, three for
+// each further box of the shape's stages and, if the unsplit tiles had an SM
+// each, four.  Band stage of one u8 pair of n x n (us), unsplit and in two or
+// three items a tile:
+//   tiles that share SMs already: 50,000 at 1,200 candidates a query 240 and 155
+//     (1 box, 4 CTAs), at 300 103 and 82, at 75 70 and 66; but 88 and 112 at 300 in 4
+//     boxes, 2 CTAs, whose two CTAs an SM gain nothing from one another
+//   tiles of an SM each: 8,000 at 3 candidates 20 and 33 (4 boxes) or 24 and 36 (1
+//     box) in three items, 20 and 22 or 24 and 22 in two, which still fit; 16,384 at
+//     1,200 92 and 112 (4 boxes), 121 and 91 (1 box, four items)
+// From two rounds of tiles the last round is full enough: 100,000 at 600 in 2 boxes,
+// 3 CTAs is 181 unsplit.
+int band_split(const Launch &L, int sms, int ctas, int boxes) {
+    const int64_t slots = ctas * (int64_t)sms;
+    if (L.ntiles >= 2 * slots) return 1;
     int best = 1;
     double least = 1e30;
     for (int s = 1; s <= kMaxSplit && (s == 1 || L.ntiles * s <= L.part_items); s++) {
-        const double t = (double)((L.ntiles * s + slots - 1) / slots) * (1.0 + L.tile_work / s);
+        double t = (double)((L.ntiles * s + slots - 1) / slots) * (1.0 + L.tile_work / s);
+        if (s > 1) t += 0.6;
+        if (s > 1 && L.ntiles * s > sms) t += 3.0 * (boxes - 1) + (L.ntiles <= sms ? 4.0 : 0.0);
         if (t < least) {
             least = t;
             best = s;
@@ -1760,7 +1766,7 @@ cudaError_t launch_band_shape(Launch L, int sms, const CUtensorMap &tA, const CU
                               bool zero_work, bool pdl, cudaStream_t s) {
     const int smem = (int)BandShape<CB, CPS, FLT>::kDynSmem;
     const int64_t slots = CPS * (int64_t)sms;
-    L.split = FLT ? 1 : band_split(L, slots);  // float rows keep up to eight candidates each for the rerank
+    L.split = FLT ? 1 : band_split(L, sms, CPS, CB);  // float rows keep up to eight candidates each for the rerank
     const int64_t grid = std::min(L.ntiles * L.split, slots);
     cudaError_t e;
     if (zero_work && (e = cudaMemsetAsync(L.work, 0, sizeof(uint32_t), s)) != cudaSuccess) return e;
