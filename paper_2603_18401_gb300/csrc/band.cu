@@ -1794,8 +1794,17 @@ cudaError_t launch_band(const Launch &L, int sms, int shape, cudaStream_t s, boo
     if (e != cudaSuccess) return e;
     if ((e = make_tmap(&tB, L.descB, flt ? L.nr : kTM, kBoxR)) != cudaSuccess) return e;
     if (flt) {
-        e = L.qcount ? launch_band_shape<1, 3, true, true>(L, sms, tA, tB, zero_work, true, s)
-                     : launch_band_shape<1, 3, true>(L, sms, tA, tB, zero_work, true, s);
+        // Two boxes to a stage where every tile has its CTA in one round of two per
+        // SM, else one box and three CTAs.  (Band stage, 2 boxes against 1, us:
+        // 20,000 x 60,000 float at 300 candidates a query 338 and 390, at 30 136 and
+        // 160; 38,000 x 38,000 at 30 110 and 111; 16 pairs of 16,384, 13.5 tiles per SM,
+        // at 30 380 and 340.)
+        if (L.ntiles <= 2 * (int64_t)sms)
+            e = L.qcount ? launch_band_shape<2, 2, true, true>(L, sms, tA, tB, zero_work, true, s)
+                         : launch_band_shape<2, 2, true>(L, sms, tA, tB, zero_work, true, s);
+        else
+            e = L.qcount ? launch_band_shape<1, 3, true, true>(L, sms, tA, tB, zero_work, true, s)
+                         : launch_band_shape<1, 3, true>(L, sms, tA, tB, zero_work, true, s);
         if (e != cudaSuccess) return e;
         const int64_t grid = std::min<int64_t>(L.ntiles, 4 * (int64_t)sms);
         return launch_pdl(rerank_kernel, dim3((unsigned)grid), dim3(kRerankThreads), 0, s, L);

@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 import synth
-from test_gpu_parity import check_candidates, mt  # noqa: F401
+from test_gpu_parity import check_candidates, check_matches, mt  # noqa: F401
 from test_gpu_tile_split import KEYS, scene
 
 pytestmark = pytest.mark.gpu
@@ -50,3 +50,24 @@ def test_several_pairs(mt):
         mt.set_params(form=0, tune=1)
     for k in KEYS:
         assert np.array_equal(got[k], ref[k]), k
+
+
+@pytest.mark.parametrize("tiles", [1, 152, 304, 305])
+@pytest.mark.parametrize("eps", [0.05, 30.0, 300.0])
+def test_floats(mt, tiles, eps):
+    """Float rows on both sides of two tiles per SM; matches and counts."""
+    sc = synth.uniform_pair(np.random.default_rng(tiles), 128 * tiles - 3, 230,
+                            synth.fundamental(*2 * [synth.intrinsics(500.0, 640, 480)],
+                                              synth.rotation([0, 1, 0], 5.0), [1.0, 0.1, 0.02]),
+                            eps=eps, kind=synth.DESC_F32_L2, dim=128)
+    d = mt.to_device(sc)
+    args = (d["xy1"], d["xy2"], d["F"], d["eps"], d["desc1"], d["desc2"], d["kind"], d["dim"], d["width"], d["height"])
+    try:
+        mt.set_params(form=2, tune=0)
+        got = {k: v.cpu().numpy() for k, v in mt.match(*args).items()}
+    finally:
+        mt.set_params(form=0, tune=1)
+    ref = check_matches(got, sc)
+    out = {k: v.cpu().numpy() for k, v in mt.match(*args, csr=True, cand_capacity=sc.m * 230).items()}
+    check_candidates(out, sc)
+    check_matches(out, sc, ref)
